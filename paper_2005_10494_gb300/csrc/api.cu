@@ -18,6 +18,7 @@
 #include "tps.cuh"
 #include "mcd_internal.cuh"
 #include "pipes.cuh"
+#include "ranked_api.cuh"
 #include "smooth.cuh"
 
 using namespace mcd;
@@ -66,6 +67,28 @@ struct SharedSeg {
     int grid = 0;
     int blocks_per_sm = 0;
 };
+
+// One round of the ranked shared-draw path: families [fam0, fam0 + n_fam) of
+// dimension d against the draws of segments [seg0, seg1).
+struct RankLaunch {
+    int d = 0, words = 0, fam_cap = 0;
+    bool sort = false;               // first round of its families
+    int fam0 = 0, n_fam = 0, seg0 = 0, seg1 = 0, item0 = 0, item1 = 0;
+    int64_t n_tiles = 0, n_units = 0;
+};
+
+// The ranked path queues three kernels and builds rows per chunk, about 20 us
+// together; the kernel that tests every design against every draw spends its
+// threads in rounds of 256 designs.  Measured on one group (forward, d = 1, 3,
+// 5, 10, 20, 32..2048 designs, 1e4..6.4e5 draws) the two cross where
+// d x draws x ceil(designs / 256) is about 1.25e6: at d = 3, 32 x 640k takes
+// 69 us there and 59 us ranked, 512 x 160k 51 and 60 us; at d = 20, 32 x 160k
+// 255 and 223 us.  The work of a dimension's groups adds up (one launch), and
+// groups of few draws do not pay for their rows.
+constexpr double kRankMinWork = 1.25e6;
+constexpr uint64_t kRankMinDraws = 16384;
+constexpr size_t kRankWorkspace = 64ull << 20;   // ranks of one round: well inside the 129 MB L2
+constexpr int kRankFamilies = 256;               // families of one round (their thresholds: 74 KB each at d=3)
 
 // Which tiles a plan keeps (the autotuner times filtered plans).
 struct TileFilter {
@@ -128,6 +151,16 @@ struct mcd_plan {
     SharedTile* d_stiles = nullptr;
     uint32_t* d_slist = nullptr;       // designs of the shared tiles, chunk by chunk
     size_t gacc_len = 0;
+    // ranked shared-draw path
+    std::vector<RankLaunch> rlaunches;
+    RankFam* d_rfams = nullptr;
+    RankSeg* d_rsegs = nullptr;
+    RankItem* d_ritems = nullptr;
+    uint32_t* d_rlist = nullptr;
+    float* d_rdistinct = nullptr;
+    int32_t* d_rndistinct = nullptr;
+    uint16_t* d_rpos = nullptr;
+    uint16_t* d_ranks = nullptr;
     std::vector<void*> owned;
     // CUDA graphs, one per launch kind (0 eval, 1 grad)
     cudaGraphExec_t gexec[2] = {nullptr, nullptr};
@@ -250,6 +283,104 @@ mcd_status validate_problem(mcd_ctx* ctx, const mcd_problem* pr, int32_t k) {
     return MCD_OK;
 }
 
+// Host tables of the ranked path and the workspace they need.
+struct RankTables {
+    std::vector<RankFam> fams;
+    std::vector<RankSeg> segs;
+    std::vector<RankItem> items;
+    std::vector<uint32_t> list;
+    size_t ws_bytes = 0, thresholds = 0, coords = 0;
+};
+
+// Families of at most rank_family(d) designs, grouped by kernel (d, words),
+// and rounds of at most kRankFamilies families and kRankWorkspace bytes of
+// ranks; a family with more draws than a round holds continues in the next.
+void rank_plan(const mcd_problem* pr, const std::vector<std::vector<int>>& groups, std::vector<RankLaunch>& launches,
+               RankTables& t) {
+    std::map<std::pair<int, int>, std::vector<int>> classes;
+    for (const std::vector<int>& g : groups) {
+        const int d = pr->scen_d[pr->design_scen[g[0]]];
+        const size_t cap = static_cast<size_t>(rank_family(d));
+        for (size_t c = 0; c < g.size(); c += cap) {
+            RankFam f;
+            f.key = pr->key[g[0]];
+            f.list_off = static_cast<uint32_t>(t.list.size());
+            f.cnt = static_cast<int32_t>(std::min(cap, g.size() - c));
+            f.scen = pr->design_scen[g[0]];
+            f.pad = 0;
+            for (int32_t q = 0; q < f.cnt; ++q) t.list.push_back(static_cast<uint32_t>(g[c + q]));
+            classes[{d, rank_words(d, f.cnt)}].push_back(static_cast<int>(t.fams.size()));
+            t.fams.push_back(f);
+        }
+    }
+    std::vector<RankFam> ordered;
+    for (const auto& cl : classes) {
+        const int d = cl.first.first, words = cl.first.second;
+        const int g = group_of(d), batch = rank_batch(d, words, nullptr), chunk = 32 * words;
+        const size_t row = 2 * static_cast<size_t>((d + 3) / 4 * 4);
+        const uint64_t cap = kRankWorkspace / row / 4096 * 4096;
+        for (size_t f0 = 0; f0 < cl.second.size(); f0 += kRankFamilies) {
+            const size_t f1 = std::min(cl.second.size(), f0 + kRankFamilies);
+            RankLaunch l;
+            l.d = d;
+            l.words = words;
+            l.sort = true;
+            l.fam0 = static_cast<int>(ordered.size());
+            l.n_fam = static_cast<int>(f1 - f0);
+            l.fam_cap = 32;
+            for (size_t q = f0; q < f1; ++q) {
+                ordered.push_back(t.fams[cl.second[q]]);
+                while (l.fam_cap < ordered.back().cnt) l.fam_cap <<= 1;
+            }
+            t.thresholds = std::max(t.thresholds, static_cast<size_t>(l.n_fam) * d * l.fam_cap);
+            t.coords = std::max(t.coords, static_cast<size_t>(l.n_fam) * d);
+            l.seg0 = l.seg1 = static_cast<int>(t.segs.size());
+            uint64_t used = 0;
+            auto close = [&]() {
+                l.seg1 = static_cast<int>(t.segs.size());
+                if (l.seg1 == l.seg0) return;
+                l.item0 = static_cast<int>(t.items.size());
+                l.n_units = 0;
+                for (int q = l.seg0; q < l.seg1; ++q) {
+                    const int nch = (ordered[t.segs[q].fam].cnt + chunk - 1) / chunk;
+                    for (int c = 0; c < nch; ++c) {
+                        t.items.push_back({l.n_units, q, c});
+                        l.n_units += (t.segs[q].n + batch - 1) / batch;
+                    }
+                }
+                l.item1 = static_cast<int>(t.items.size());
+                t.ws_bytes = std::max(t.ws_bytes, static_cast<size_t>(used) * row);
+                launches.push_back(l);
+                l.sort = false;
+                l.seg0 = l.seg1;
+                l.n_tiles = 0;
+                used = 0;
+            };
+            for (int f = l.fam0; f < l.fam0 + l.n_fam; ++f) {
+                const int j0 = static_cast<int>(t.list[ordered[f].list_off]);
+                const uint64_t begin = pr->draw_begin ? pr->draw_begin[j0] : 0, n = pr->n_draws[j0];
+                for (uint64_t at = 0; at < n;) {
+                    if (used + 4096 > cap) close();
+                    const uint64_t take = std::min<uint64_t>(n - at, cap - used);
+                    RankSeg sg;
+                    sg.start = begin + at;
+                    sg.n = static_cast<uint32_t>(take);
+                    sg.fam = f;
+                    sg.ws_off = used;
+                    sg.tile0 = l.n_tiles;
+                    const uint64_t groups_n = (sg.start % g + take + g - 1) / g;
+                    l.n_tiles += static_cast<int64_t>((groups_n + kRankDrawThreads - 1) / kRankDrawThreads);
+                    t.segs.push_back(sg);
+                    at += take;
+                    used += (take + 3) / 4 * 4;
+                }
+            }
+            close();
+        }
+    }
+    t.fams.swap(ordered);
+}
+
 // Host-side planning: tiles, batch slots, offsets; uploads; workspace.
 // The filter keeps only some designs' tiles (the autotuner's timing plans).
 mcd_status plan_build(mcd_ctx* ctx, const mcd_problem* pr, int32_t flags, int32_t k, mcd_plan* pl,
@@ -270,7 +401,7 @@ mcd_status plan_build(mcd_ctx* ctx, const mcd_problem* pr, int32_t flags, int32_
 
     // common-random-number groups for the shared-draw kernel
     std::vector<char> is_shared(J, 0);
-    std::vector<std::vector<int>> groups;
+    std::vector<std::vector<int>> groups, rgroups;       // shared-draw kernel, ranked path
     if (flags & MCD_PLAN_SHARED) {
         if (pl->fp64) return fail(ctx, MCD_EUNSUPPORTED, "MCD_PLAN_SHARED is not available with MCD_PLAN_FP64");
         std::map<std::tuple<int, uint64_t, uint64_t, uint64_t>, std::vector<int>> by;
@@ -279,10 +410,19 @@ mcd_status plan_build(mcd_ctx* ctx, const mcd_problem* pr, int32_t flags, int32_
             if (pr->n_draws[j] == 0) continue;
             by[std::make_tuple(pr->design_scen[j], pr->key[j], begin, pr->n_draws[j])].push_back(j);
         }
+        std::vector<double> rank_work(MCD_MAX_D + 1, 0.0);
+        for (auto& kv : by) {
+            const uint64_t n = std::get<3>(kv.first);
+            const int d = pr->scen_d[std::get<0>(kv.first)];
+            if (static_cast<int>(kv.second.size()) >= MCD_SHARED_MIN && n >= kRankMinDraws)
+                rank_work[d] += static_cast<double>(d) * static_cast<double>(n) * static_cast<double>((kv.second.size() + 255) / 256);
+        }
         for (auto& kv : by) {
             if (static_cast<int>(kv.second.size()) < MCD_SHARED_MIN) continue;
             for (int j : kv.second) is_shared[j] = 1;
-            groups.push_back(std::move(kv.second));
+            const bool ranked = !grad_kernel && std::get<3>(kv.first) >= kRankMinDraws &&
+                                rank_work[pr->scen_d[std::get<0>(kv.first)]] >= kRankMinWork;
+            (ranked ? rgroups : groups).push_back(std::move(kv.second));
         }
     }
 
@@ -392,6 +532,9 @@ mcd_status plan_build(mcd_ctx* ctx, const mcd_problem* pr, int32_t flags, int32_
             max_tiles = std::max<int64_t>(max_tiles, static_cast<int64_t>((n_draws[j0] + T - 1) / T));
         }
     }
+    RankTables rt;
+    pl->rlaunches.clear();
+    rank_plan(pr, rgroups, pl->rlaunches, rt);
     if (total_tiles >= (1ll << 31)) return fail(ctx, MCD_EINVAL, "too many tiles (reduce n_draws)");
     pl->n_tiles = total_tiles;
     pl->batches = static_cast<int>(std::min<int64_t>(kMaxBatches, max_tiles));
@@ -488,6 +631,7 @@ mcd_status plan_build(mcd_ctx* ctx, const mcd_problem* pr, int32_t flags, int32_
         }
     }
     pl->n_shared_tiles = static_cast<int64_t>(stiles.size());
+    for (const RankLaunch& l : pl->rlaunches) pl->n_shared_tiles += l.n_units;
 
     // by segment, and within a segment the costliest tiles first: the
     // dynamic ticket then leaves only small tiles for the tail
@@ -524,6 +668,20 @@ mcd_status plan_build(mcd_ctx* ctx, const mcd_problem* pr, int32_t flags, int32_
     if ((st = plan_alloc(pl, &pl->d_stiles, stiles.size())) != MCD_OK) return st;
     if ((st = plan_alloc(pl, &pl->d_slist, slist.size())) != MCD_OK) return st;
     if (grad_kernel && (st = plan_alloc(pl, &pl->d_gacc, pl->gacc_len)) != MCD_OK) return st;
+    if (!pl->rlaunches.empty()) {
+        if ((st = plan_alloc(pl, &pl->d_rfams, rt.fams.size())) != MCD_OK) return st;
+        if ((st = plan_alloc(pl, &pl->d_rsegs, rt.segs.size())) != MCD_OK) return st;
+        if ((st = plan_alloc(pl, &pl->d_ritems, rt.items.size())) != MCD_OK) return st;
+        if ((st = plan_alloc(pl, &pl->d_rlist, rt.list.size())) != MCD_OK) return st;
+        if ((st = plan_alloc(pl, &pl->d_rdistinct, rt.thresholds)) != MCD_OK) return st;
+        if ((st = plan_alloc(pl, &pl->d_rpos, rt.thresholds)) != MCD_OK) return st;
+        if ((st = plan_alloc(pl, &pl->d_rndistinct, rt.coords)) != MCD_OK) return st;
+        if ((st = plan_alloc(pl, &pl->d_ranks, rt.ws_bytes / sizeof(uint16_t))) != MCD_OK) return st;
+        if ((st = plan_upload(pl, pl->d_rfams, rt.fams)) != MCD_OK) return st;
+        if ((st = plan_upload(pl, pl->d_rsegs, rt.segs)) != MCD_OK) return st;
+        if ((st = plan_upload(pl, pl->d_ritems, rt.items)) != MCD_OK) return st;
+        if ((st = plan_upload(pl, pl->d_rlist, rt.list)) != MCD_OK) return st;
+    }
 
     if ((st = plan_upload(pl, pl->d_designs, designs)) != MCD_OK) return st;
     if ((st = plan_upload(pl, pl->d_tiles, tiles)) != MCD_OK) return st;
@@ -554,7 +712,8 @@ mcd_status plan_build(mcd_ctx* ctx, const mcd_problem* pr, int32_t flags, int32_
     return MCD_OK;
 }
 
-void fill_round_keys(uint64_t seed, SampleParams& sp) {
+template <typename Params>
+void fill_round_keys(uint64_t seed, Params& sp) {
     for (int r = 0; r < 10; ++r) {
         sp.rk0[r] = static_cast<uint32_t>(seed) + static_cast<uint32_t>(r) * kPhiloxW0;
         sp.rk1[r] = static_cast<uint32_t>(seed >> 32) + static_cast<uint32_t>(r) * kPhiloxW1;
@@ -633,6 +792,39 @@ mcd_status enqueue(mcd_plan* pl, const LaunchArgs& a, cudaStream_t stream) {
         sp.ticket = pl->d_ticket + pl->segs.size() + q;
         MCD_CUDA(launch_shared(sg.d, a.grad, sp, pl->d_stiles + sg.tile_begin, pl->d_slist, sg.grid, stream),
                  "shared-draw launch");
+    }
+    for (const RankLaunch& l : pl->rlaunches) {
+        RankParams rp;
+        std::memset(&rp, 0, sizeof(rp));
+        rp.fams = pl->d_rfams;
+        rp.segs = pl->d_rsegs;
+        rp.items = pl->d_ritems;
+        rp.list = pl->d_rlist;
+        rp.designs = pl->d_designs;
+        rp.mu = pl->mu;
+        rp.b = pl->b;
+        rp.L32 = pl->d_L32;
+        rp.L_off = pl->d_L_off;
+        rp.scen_ok = pl->d_scen_ok;
+        rp.distinct = pl->d_rdistinct;
+        rp.n_distinct = pl->d_rndistinct;
+        rp.pos = pl->d_rpos;
+        rp.ranks = pl->d_ranks;
+        rp.hits = pl->d_hits;
+        rp.status = ctx->d_status;
+        rp.n_tiles = l.n_tiles;
+        rp.n_units = l.n_units;
+        rp.fam_cap = l.fam_cap;
+        rp.fam0 = l.fam0;
+        rp.n_fam = l.n_fam;
+        rp.seg0 = l.seg0;
+        rp.seg1 = l.seg1;
+        rp.item0 = l.item0;
+        rp.item1 = l.item1;
+        fill_round_keys(a.seed, rp);
+        if (l.sort) MCD_CUDA(launch_rank_sort(l.d, rp, stream), "threshold sort launch");
+        MCD_CUDA(launch_rank_draws(l.d, rp, ctx->sm_count, stream), "ranked draws launch");
+        MCD_CUDA(launch_rank_count(l.d, l.words, rp, ctx->sm_count, stream), "ranked count launch");
     }
     for (size_t q = 0; q < pl->segs.size(); ++q) {
         const Segment& sg = pl->segs[q];
@@ -930,6 +1122,15 @@ mcd_status mcd_plan_config(const mcd_plan* plan, int32_t d, int32_t* threads, in
             if (threads) *threads = kSharedThreads;
             if (tile_draws) *tile_draws = sg.tile_draws;
             if (blocks_per_sm) *blocks_per_sm = sg.blocks_per_sm;
+            return MCD_OK;
+        }
+        for (const RankLaunch& l : plan->rlaunches) {
+            if (l.d != d) continue;
+            int th = 0;
+            const int batch = rank_batch(d, l.words, &th);
+            if (threads) *threads = th;
+            if (tile_draws) *tile_draws = batch;
+            if (blocks_per_sm) *blocks_per_sm = 1;
             return MCD_OK;
         }
         return MCD_EINVAL;
