@@ -55,71 +55,106 @@ __device__ inline int basis(double dx, double dy, int degree, bool two_d, double
     return n;
 }
 
-// One thread per class pair: stencil weights w[(dx+R)(2R+1) + (dy+R)] in FP64.
+// Stencil weights w[(dx+R)(2R+1) + (dy+R)] of one class pair per block, in FP64.
 // Class of a position: lo = min(i, R) points below, hi = min(G-1-i, R) above;
 // class id = lo (R+1) + hi.  1-D grids use only the x axis (classes in x).
-__global__ void weights_kernel(int R, double bw, int degree, bool two_d, int gx, int gy,
-                               double* w64, float* w32, DevStatus* status) {
+// A thread per entry of the normal matrix M sums over the window, the
+// elimination takes a row per thread, and a thread per tap writes the stencil;
+// every entry sees its operations in the order of the sequential solve.  One
+// thread per class pair spent 116 us in chains of FP64 operations, whatever the
+// grid; FP64 latency of one such chain per pivot is what is left.
+constexpr int kWeightThreads = 64;
+__global__ void __launch_bounds__(kWeightThreads) weights_kernel(int R, double bw, int degree, bool two_d, int gx, int gy,
+                                                                 double* w64, float* w32, DevStatus* status) {
+    __shared__ double sM[6][7];            // normal matrix, right-hand side e_0 in column 6
+    __shared__ double sW[kMaxReach + 1];   // tricube weights of |dx|
+    __shared__ double su[6];
     const int ncls = (R + 1) * (R + 1);
-    const int id = blockIdx.x * blockDim.x + threadIdx.x;
-    if (id >= (two_d ? ncls * ncls : ncls)) return;
+    const int id = blockIdx.x, tid = threadIdx.x;
     const int cx = two_d ? id / ncls : id, cy = two_d ? id % ncls : 0;
     const int xlo = cx / (R + 1), xhi = cx % (R + 1);
     const int ylo = two_d ? cy / (R + 1) : 0, yhi = two_d ? cy % (R + 1) : 0;
     const int T = 2 * R + 1;
     double* w = w64 + static_cast<int64_t>(id) * kMaxTaps;
     float* wf = w32 + static_cast<int64_t>(id) * kMaxTaps;
-    // the thread of the interior class pair also fills the compact copy
+    // the block of the interior class pair also fills the compact copy
     // (zeros when this grid has no interior point)
     float* wint = (xlo == R && xhi == R && (!two_d || (ylo == R && yhi == R)))
                       ? w32 + static_cast<int64_t>(kClassSlots) * kMaxTaps : nullptr;
-    for (int q = 0; q < kMaxTaps; ++q) { w[q] = 0.0; wf[q] = 0.0f; }
+    for (int q = tid; q < kMaxTaps; q += kWeightThreads) { w[q] = 0.0; wf[q] = 0.0f; }
     if (wint)
-        for (int q = 0; q < kIntSlot; ++q) wint[q] = 0.0f;
+        for (int q = tid; q < kIntSlot; q += kWeightThreads) wint[q] = 0.0f;
     // classes that no position of this grid has are skipped
     if (xlo + xhi + 1 > gx || (xlo < R && xhi < R && xlo + xhi + 1 != gx)) return;
     if (two_d && (ylo + yhi + 1 > gy || (ylo < R && yhi < R && ylo + yhi + 1 != gy))) return;
-    double M[6][6] = {};
+    if (tid <= R) sW[tid] = tricube(tid / bw);
+    __syncthreads();
     double x[6];
-    int nb = 0;
-    for (int dx = -xlo; dx <= xhi; ++dx) {
-        for (int dy = -ylo; dy <= yhi; ++dy) {
-            const double W = tricube(dx / bw) * (two_d ? tricube(dy / bw) : 1.0);
-            nb = basis(dx, dy, degree, two_d, x);
-            for (int a = 0; a < nb; ++a)
-                for (int c = 0; c < nb; ++c) M[a][c] += W * x[a] * x[c];
+    const int nb = basis(0.0, 0.0, degree, two_d, x);
+    if (tid < 36) {
+        const int a = tid / 6, c = tid % 6;
+        double m = 0.0;
+        for (int dx = -xlo; dx <= xhi; ++dx) {
+            for (int dy = -ylo; dy <= yhi; ++dy) {
+                const double W = sW[abs(dx)] * (two_d ? sW[abs(dy)] : 1.0);
+                basis(dx, dy, degree, two_d, x);
+                double xa = 0.0, xc = 0.0;
+#pragma unroll
+                for (int e = 0; e < 6; ++e) {
+                    if (e == a) xa = x[e];
+                    if (e == c) xc = x[e];
+                }
+                if (a < nb && c < nb) m += W * xa * xc;
+            }
         }
+        sM[a][c] = m;
+        if (c == 0) sM[a][6] = a == 0 ? 1.0 : 0.0;
     }
+    __syncthreads();
     // u = M^-1 e_0 by Gaussian elimination with partial pivoting
-    double u[6] = {1.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     for (int col = 0; col < nb; ++col) {
         int piv = col;
-        for (int r = col + 1; r < nb; ++r) if (fabs(M[r][col]) > fabs(M[piv][col])) piv = r;
-        if (!(fabs(M[piv][col]) > 1e-12)) { set_status(status, MCD_EINVAL, id); return; }
-        if (piv != col) {
-            for (int c = 0; c < nb; ++c) { const double tmp = M[col][c]; M[col][c] = M[piv][c]; M[piv][c] = tmp; }
-            const double tu = u[col]; u[col] = u[piv]; u[piv] = tu;
+        for (int r = col + 1; r < nb; ++r) if (fabs(sM[r][col]) > fabs(sM[piv][col])) piv = r;
+        if (!(fabs(sM[piv][col]) > 1e-12)) {             // the same for every thread
+            if (tid == 0) set_status(status, MCD_EINVAL, id);
+            return;
         }
-        for (int r = 0; r < nb; ++r) {
-            if (r == col) continue;
-            const double f = M[r][col] / M[col][col];
-            if (f == 0.0) continue;
-            for (int c = col; c < nb; ++c) M[r][c] -= f * M[col][c];
-            u[r] -= f * u[col];
+        __syncthreads();
+        if (piv != col && tid < 7) {
+            const double t = sM[col][tid];
+            sM[col][tid] = sM[piv][tid];
+            sM[piv][tid] = t;
         }
+        __syncthreads();
+        const int r = tid / 8, c = tid % 8;               // row r, column c (6: right-hand side)
+        double f = 0.0, v = 0.0;
+        const bool on = r < nb && r != col && c < 7;
+        if (on) {
+            f = sM[r][col] / sM[col][col];
+            v = sM[r][c] - f * sM[col][c];
+        }
+        __syncthreads();
+        if (on && f != 0.0 && ((c >= col && c < nb) || c == 6)) sM[r][c] = v;
+        __syncthreads();
     }
-    for (int r = 0; r < nb; ++r) u[r] /= M[r][r];
-    for (int dx = -xlo; dx <= xhi; ++dx) {
-        for (int dy = -ylo; dy <= yhi; ++dy) {
-            const double W = tricube(dx / bw) * (two_d ? tricube(dy / bw) : 1.0);
-            basis(dx, dy, degree, two_d, x);
-            double s = 0.0;
-            for (int a = 0; a < nb; ++a) s += x[a] * u[a];
-            const int q = two_d ? (dx + R) * T + (dy + R) : (dx + R);
-            w[q] = W * s;
-            wf[q] = static_cast<float>(W * s);
-            if (wint) wint[q] = wf[q];
-        }
+    if (tid < 6) su[tid] = tid < nb ? sM[tid][6] / sM[tid][tid] : 0.0;
+    __syncthreads();
+    double u[6];
+#pragma unroll
+    for (int a = 0; a < 6; ++a) u[a] = su[a];
+    const int nx = xlo + xhi + 1, ny = ylo + yhi + 1;
+    for (int t = tid; t < nx * ny; t += kWeightThreads) {
+        const int dx = t / ny - xlo, dy = t % ny - ylo;
+        const double W = sW[abs(dx)] * (two_d ? sW[abs(dy)] : 1.0);
+        basis(dx, dy, degree, two_d, x);
+        double s = 0.0;
+#pragma unroll
+        for (int a = 0; a < 6; ++a)
+            if (a < nb) s += x[a] * u[a];
+        const int q = two_d ? (dx + R) * T + (dy + R) : (dx + R);
+        w[q] = W * s;
+        wf[q] = static_cast<float>(W * s);
+        if (wint) wint[q] = wf[q];
     }
     // The interior stencil in 2-D is separable into two rank-one parts.  With
     // symmetric product weights W(dx) W(dy), the coefficients of the odd
@@ -129,10 +164,11 @@ __global__ void weights_kernel(int R, double bw, int degree, bool two_d, int gx,
     // The tile kernel applies it as two row filters (W(v), v^2 W(v)) and one
     // column pass with the weights W(u) (u_0 + u_x u^2) and W(u) u_y; for
     // degree 0 and 1, u_x = u_y = 0 (one rank-one part).
-    if (wint && two_d) {
+    if (wint && two_d && tid <= R) {
         const double ux = nb == 6 ? u[3] : 0.0, uy = nb == 6 ? u[5] : 0.0;
-        for (int k = 0; k <= R; ++k) {
-            const double wk = tricube(k / bw);
+        {
+            const int k = tid;
+            const double wk = sW[k];
             wint[kSepOff + k] = static_cast<float>(wk);
             wint[kSepOff + 4 + k] = static_cast<float>(k * k * wk);
             wint[kSepOff + 8 + k] = static_cast<float>(wk * (u[0] + ux * k * k));
@@ -826,7 +862,7 @@ cudaError_t smooth_argmax_t(int n_scen, int g1, int g2, const Elem* value, doubl
     const int ncls = (R + 1) * (R + 1);
     const int nw = two_d ? ncls * ncls : ncls;
     const int gx = two_d ? g1 : g1 * g2;
-    weights_kernel<<<(nw + 63) / 64, 64, 0, stream>>>(R, bandwidth, degree, two_d, gx, g2, wbuf, wbuf32,
+    weights_kernel<<<nw, kWeightThreads, 0, stream>>>(R, bandwidth, degree, two_d, gx, g2, wbuf, wbuf32,
                                                       status);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
