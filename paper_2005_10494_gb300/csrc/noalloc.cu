@@ -21,6 +21,7 @@
 #include <cstring>
 #include <mutex>
 
+#include "chol.cuh"
 #include "mcd_internal.cuh"
 #include "sample.cuh"
 
@@ -49,23 +50,9 @@ int g_blocks_per_sm[64][kMaxD + 1] = {};
 std::mutex g_scratch_mu;
 
 // Sigma = L L^T for the one scenario (FP64, lower triangle read), FP32 copy.
-__global__ void noalloc_cholesky_kernel(const double* __restrict__ Sigma, int d, NoAllocScratch* sc) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    bool good = true;
-    for (int i = 0; i < d && good; ++i) {
-        for (int j = 0; j <= i; ++j) {
-            double sum = Sigma[i * d + j];
-            for (int k = 0; k < j; ++k) sum -= sc->L64[i * (i + 1) / 2 + k] * sc->L64[j * (j + 1) / 2 + k];
-            if (i == j) {
-                if (!(sum > 0.0) || !isfinite(sum)) { good = false; break; }
-                sc->L64[i * (i + 1) / 2 + i] = sqrt(sum);
-            } else {
-                sc->L64[i * (i + 1) / 2 + j] = sum / sc->L64[j * (j + 1) / 2 + j];
-            }
-        }
-    }
-    for (int q = 0; q < d * (d + 1) / 2; ++q) sc->L32[q] = static_cast<float>(sc->L64[q]);
-    sc->ok = good ? 1 : 0;
+__global__ void __launch_bounds__(32) noalloc_cholesky_kernel(const double* __restrict__ Sigma, int d, NoAllocScratch* sc) {
+    const bool good = warp_factor(Sigma, d, sc->L64, sc->L32);
+    if (threadIdx.x == 0) sc->ok = good ? 1 : 0;
 }
 
 // Persistent sampling over tiles numbered design-major: tile t covers draws

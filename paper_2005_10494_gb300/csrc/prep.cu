@@ -4,6 +4,7 @@
 #include <cmath>
 #include <cstdint>
 
+#include "chol.cuh"
 #include "mcd_internal.cuh"
 #include "rng.cuh"
 
@@ -13,37 +14,21 @@ namespace {
 
 __device__ __forceinline__ int tri(int i, int j) { return i * (i + 1) / 2 + j; }
 
-// Sigma_s = L L^T (Cholesky-Banachiewicz, FP64, lower triangle of Sigma read).
-__global__ void cholesky_kernel(const double* __restrict__ Sigma, const int64_t* __restrict__ sig_off,
-                                const int32_t* __restrict__ scen_d, const int64_t* __restrict__ L_off,
-                                int n_scen, float* __restrict__ L32, double* __restrict__ L64,
-                                int32_t* __restrict__ scen_ok, DevStatus* status) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+// Sigma_s = L L^T, a warp per scenario.
+constexpr int kCholWarps = 2;
+__global__ void __launch_bounds__(32 * kCholWarps) cholesky_kernel(const double* __restrict__ Sigma,
+                                                                   const int64_t* __restrict__ sig_off,
+                                                                   const int32_t* __restrict__ scen_d,
+                                                                   const int64_t* __restrict__ L_off, int n_scen,
+                                                                   float* __restrict__ L32, double* __restrict__ L64,
+                                                                   int32_t* __restrict__ scen_ok, DevStatus* status) {
+    const int s = blockIdx.x * kCholWarps + (threadIdx.x >> 5);
     if (s >= n_scen) return;
-    const int d = scen_d[s];
-    const double* A = Sigma + sig_off[s];
-    double* L = L64 + L_off[s];
-    float* Lf = L32 + L_off[s];
-    bool good = true;
-    for (int i = 0; i < d && good; ++i) {
-        for (int j = 0; j <= i; ++j) {
-            double sum = A[i * d + j];
-            for (int k = 0; k < j; ++k) sum -= L[tri(i, k)] * L[tri(j, k)];
-            if (i == j) {
-                if (!(sum > 0.0) || !isfinite(sum)) { good = false; break; }
-                L[tri(i, i)] = sqrt(sum);
-            } else {
-                L[tri(i, j)] = sum / L[tri(j, j)];
-            }
-        }
+    const bool good = warp_factor(Sigma + sig_off[s], scen_d[s], L64 + L_off[s], L32 + L_off[s]);
+    if ((threadIdx.x & 31) == 0) {
+        scen_ok[s] = good ? 1 : 0;
+        if (!good) set_status(status, MCD_ENOTSPD, s);
     }
-    const int n = d * (d + 1) / 2;
-    for (int i = 0; i < n; ++i) {
-        if (!good) L[i] = 0.0;
-        Lf[i] = static_cast<float>(L[i]);
-    }
-    scen_ok[s] = good ? 1 : 0;
-    if (!good) set_status(status, MCD_ENOTSPD, s);
 }
 
 __device__ __forceinline__ double fix_to_double(unsigned long long v) {
@@ -188,8 +173,7 @@ __global__ void debug_normals_kernel(uint64_t seed, uint64_t key, uint64_t m_beg
 cudaError_t launch_cholesky(const double* Sigma, const int64_t* sig_off, const int32_t* scen_d,
                             const int64_t* L_off, int n_scen, float* L32, double* L64,
                             int32_t* scen_ok, DevStatus* status, cudaStream_t stream) {
-    const int threads = 64;
-    cholesky_kernel<<<(n_scen + threads - 1) / threads, threads, 0, stream>>>(
+    cholesky_kernel<<<(n_scen + kCholWarps - 1) / kCholWarps, 32 * kCholWarps, 0, stream>>>(
         Sigma, sig_off, scen_d, L_off, n_scen, L32, L64, scen_ok, status);
     return cudaGetLastError();
 }
