@@ -14,6 +14,7 @@
 
 #include <nvtx3/nvToolsExt.h>
 
+#include "finalize.cuh"
 #include "fwer.cuh"
 #include "tps.cuh"
 #include "mcd_internal.cuh"
@@ -131,6 +132,7 @@ struct mcd_plan {
     std::vector<SharedSeg> ssegs;    // shared-draw launches, after the per-design ones
     int64_t n_shared_tiles = 0;
     int batches = 1;
+    uint32_t dims = 0;               // bit d: some design has dimension d
     const double* Sigma = nullptr;
     const double* mu = nullptr;
     const double* b = nullptr;
@@ -397,6 +399,8 @@ mcd_status plan_build(mcd_ctx* ctx, const mcd_problem* pr, int32_t flags, int32_
     pl->mu = pr->mu;
     pl->b = pr->b;
     const int S = pl->S, J = pl->J;
+    pl->dims = 0;
+    for (int j = 0; j < J; ++j) pl->dims |= 1u << pr->scen_d[pr->design_scen[j]];
     const bool grad_kernel = (flags & MCD_PLAN_GRAD) != 0;
 
     // common-random-number groups for the shared-draw kernel
@@ -859,7 +863,7 @@ mcd_status enqueue(mcd_plan* pl, const LaunchArgs& a, cudaStream_t stream) {
     fp.g_lr = a.g_lr;
     fp.g_sig = a.g_sig;
     fp.g_se = a.g_se;
-    MCD_CUDA(launch_finalize(fp, a.grad, stream), "finalize launch");
+    MCD_CUDA(a.grad ? launch_finalize_grad(fp, pl->dims, stream) : launch_finalize(fp, false, stream), "finalize launch");
     return MCD_OK;
 }
 
