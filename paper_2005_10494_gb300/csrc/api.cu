@@ -88,6 +88,11 @@ struct RankLaunch {
 // groups of few draws do not pay for their rows.
 constexpr double kRankMinWork = 1.25e6;
 constexpr uint64_t kRankMinDraws = 16384;
+
+// Blocks per SM for which the tiles of shared draws of a gradient plan are sized.
+// They fix which draws are summed in FP32 before the fixed-point sums, and which
+// share a batch slot, so results do not move with a kernel's register count.
+constexpr int kTileBlocks[MCD_MAX_D + 1] = {0, 4, 3, 3, 2, 2, 2, 2, 2, 2, 2, 2, 2, 1, 2, 1, 2, 1, 2, 1, 2};
 constexpr size_t kRankWorkspace = 64ull << 20;   // ranks of one round: well inside the 129 MB L2
 constexpr int kRankFamilies = 256;               // families of one round (their thresholds: 74 KB each at d=3)
 
@@ -524,7 +529,7 @@ mcd_status plan_build(mcd_ctx* ctx, const mcd_problem* pr, int32_t flags, int32_
             if (e != cudaSuccess) return cuda_fail(ctx, e, "occupancy query");
             sg.blocks_per_sm = std::max(1, bps);
             const double bd = shared_batch_draws(d);
-            const double want = chunk_draws[d] / (16.0 * ctx->sm_count * sg.blocks_per_sm);
+            const double want = chunk_draws[d] / (16.0 * ctx->sm_count * (grad_kernel ? kTileBlocks[d] : sg.blocks_per_sm));
             const int64_t mult = std::max<int64_t>(1, std::min<int64_t>(256, std::llround(want / bd)));
             sg.tile_draws = mult * static_cast<int64_t>(bd);
             stile_draws[d] = sg.tile_draws;

@@ -1,12 +1,12 @@
 // Shared-draw kernels of d = 1..10.
-#include "shared.cuh"
+#include "boxed.cuh"
 
 namespace mcd {
 
 #define MCD_SHARED_CASE(D) \
     case D: *smem = grad ? shared_smem<D, true>() : shared_smem<D, false>(); \
             *dpt = grad ? SharedShape<D, true>::kDpt : SharedShape<D, false>::kDpt; \
-            return grad ? shared_fn<D, true>() : shared_fn<D, false>();
+            return grad ? adjoint_fn<D>() : shared_fn<D, false>();
 
 const void* shared_kernel_a(int d, bool grad, size_t* smem, int* dpt) {
     switch (d) {
