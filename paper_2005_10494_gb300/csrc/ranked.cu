@@ -178,11 +178,29 @@ cudaError_t launch_rank_sort(int d, const RankParams& p, cudaStream_t stream) {
     return cudaGetLastError();
 }
 
+namespace {
+
+// Dynamic shared memory of the two kernels for families of up to `cap` designs.
+size_t draws_smem(int d, int cap) { return static_cast<size_t>(d) * cap * sizeof(float); }
+size_t count_smem(const RankKernels& k, int d, int cap) {
+    return k.count_rows + static_cast<size_t>(d) * (cap / 32 + 1) * 8;
+}
+
+// The limit is a property of the function, common to every context and thread,
+// so it is always written with the same value: what the largest family needs
+// (106 KB and 218 KB at most).  A value per launch let a thread with small
+// families lower it between another's call here and its launch, which then failed.
+cudaError_t set_limit(const void* fn, size_t largest) {
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(largest));
+}
+
+}  // namespace
+
 cudaError_t launch_rank_draws(int d, const RankParams& p, int sms, cudaStream_t stream) {
     RankKernels k;
     if (!select_rank(d, 4, &k)) return cudaErrorInvalidValue;
-    const size_t smem = static_cast<size_t>(d) * p.fam_cap * sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(k.draws, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    const size_t smem = draws_smem(d, p.fam_cap);
+    cudaError_t e = set_limit(k.draws, draws_smem(d, rank_family(d)));
     if (e != cudaSuccess) return e;
     int bps = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k.draws, kRankDrawThreads, smem)) != cudaSuccess) return e;
@@ -194,8 +212,8 @@ cudaError_t launch_rank_draws(int d, const RankParams& p, int sms, cudaStream_t 
 cudaError_t launch_rank_count(int d, int words, const RankParams& p, int sms, cudaStream_t stream) {
     RankKernels k;
     if (!select_rank(d, words, &k)) return cudaErrorInvalidValue;
-    const size_t smem = k.count_rows + static_cast<size_t>(d) * (p.fam_cap / 32 + 1) * 8;
-    cudaError_t e = cudaFuncSetAttribute(k.count, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    const size_t smem = count_smem(k, d, p.fam_cap);
+    cudaError_t e = set_limit(k.count, count_smem(k, d, rank_family(d)));
     if (e != cudaSuccess) return e;
     int bps = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k.count, k.threads, smem)) != cudaSuccess) return e;
