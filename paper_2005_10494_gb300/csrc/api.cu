@@ -541,9 +541,6 @@ mcd_status plan_build(mcd_ctx* ctx, const mcd_problem* pr, int32_t flags, int32_
             max_tiles = std::max<int64_t>(max_tiles, static_cast<int64_t>((n_draws[j0] + T - 1) / T));
         }
     }
-    RankTables rt;
-    pl->rlaunches.clear();
-    rank_plan(pr, rgroups, pl->rlaunches, rt);
     if (total_tiles >= (1ll << 31)) return fail(ctx, MCD_EINVAL, "too many tiles (reduce n_draws)");
     pl->n_tiles = total_tiles;
     pl->batches = static_cast<int>(std::min<int64_t>(kMaxBatches, max_tiles));
@@ -567,6 +564,26 @@ mcd_status plan_build(mcd_ctx* ctx, const mcd_problem* pr, int32_t flags, int32_
                 return fail(ctx, MCD_EINVAL, "n_draws too large for a gradient plan (2^32 draws per batch slot, 32 slots)", j0);
         }
     }
+    // Refused before any table is built.  A ranked group counts as the tiles of
+    // 256 batches that the shared-draw kernel would take, so that both paths
+    // refuse the same draw counts.
+    {
+        double tiles = static_cast<double>(total_tiles);
+        for (const SChunk& c : chunks) {
+            const int j0 = groups[c.g][0];
+            tiles += std::ceil(static_cast<double>(n_draws[j0]) / static_cast<double>(stile_draws[scen_d[pr->design_scen[j0]]]));
+        }
+        for (const std::vector<int>& g : rgroups) {
+            const int d = scen_d[pr->design_scen[g[0]]];
+            const size_t cap = static_cast<size_t>(kSharedThreads) * shared_designs_per_thread(d, false);
+            tiles += static_cast<double>((g.size() + cap - 1) / cap) *
+                     std::ceil(static_cast<double>(n_draws[g[0]]) / (256.0 * shared_batch_draws(d)));
+        }
+        if (tiles >= 2147483648.0) return fail(ctx, MCD_EINVAL, "too many tiles (reduce n_draws)");
+    }
+    RankTables rt;
+    pl->rlaunches.clear();
+    rank_plan(pr, rgroups, pl->rlaunches, rt);
     for (int j = 0; j < J; ++j) designs[j].acc_off = 3 * designs[j].vec_off * B;
     pl->gacc_len = static_cast<size_t>(3) * vo * B;
 
@@ -622,8 +639,6 @@ mcd_status plan_build(mcd_ctx* ctx, const mcd_problem* pr, int32_t flags, int32_
             for (int bb = 0; bb < B; ++bb)
                 batch_draws[static_cast<size_t>(gr[c.first + q]) * B + bb] += chunk_batch[static_cast<size_t>(bb)];
     }
-    if (static_cast<int64_t>(stiles.size()) + total_tiles >= (1ll << 31))
-        return fail(ctx, MCD_EINVAL, "too many tiles (reduce n_draws)");
     std::stable_sort(stiles.begin(), stiles.end(), [&](const SharedTile& a, const SharedTile& c) {
         const int da = scen_d[a.scen], dc = scen_d[c.scen];
         if (da != dc) return da < dc;
