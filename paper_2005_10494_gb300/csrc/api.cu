@@ -137,7 +137,7 @@ struct mcd_plan {
     std::vector<SharedSeg> ssegs;    // shared-draw launches, after the per-design ones
     int64_t n_shared_tiles = 0;
     int batches = 1;
-    uint32_t dims = 0;               // bit d: some design has dimension d
+    FinalizeDims fdims = {};         // the designs by dimension (gradient plans)
     const double* Sigma = nullptr;
     const double* mu = nullptr;
     const double* b = nullptr;
@@ -404,8 +404,6 @@ mcd_status plan_build(mcd_ctx* ctx, const mcd_problem* pr, int32_t flags, int32_
     pl->mu = pr->mu;
     pl->b = pr->b;
     const int S = pl->S, J = pl->J;
-    pl->dims = 0;
-    for (int j = 0; j < J; ++j) pl->dims |= 1u << pr->scen_d[pr->design_scen[j]];
     const bool grad_kernel = (flags & MCD_PLAN_GRAD) != 0;
 
     // common-random-number groups for the shared-draw kernel
@@ -691,7 +689,22 @@ mcd_status plan_build(mcd_ctx* ctx, const mcd_problem* pr, int32_t flags, int32_
         return st;
     if ((st = plan_alloc(pl, &pl->d_stiles, stiles.size())) != MCD_OK) return st;
     if ((st = plan_alloc(pl, &pl->d_slist, slist.size())) != MCD_OK) return st;
-    if (grad_kernel && (st = plan_alloc(pl, &pl->d_gacc, pl->gacc_len)) != MCD_OK) return st;
+    if (grad_kernel) {
+        if ((st = plan_alloc(pl, &pl->d_gacc, pl->gacc_len)) != MCD_OK) return st;
+        pl->fdims = FinalizeDims{};
+        for (int j = 0; j < J; ++j) ++pl->fdims.first[designs[j].d];
+        const bool mixed = J > 0 && pl->fdims.first[designs[0].d] < J;
+        for (int d = 1; d <= MCD_MAX_D; ++d) pl->fdims.first[d] += pl->fdims.first[d - 1];
+        if (mixed) {
+            std::vector<uint32_t> order(J);
+            std::vector<int32_t> at(pl->fdims.first, pl->fdims.first + MCD_MAX_D + 1);
+            for (int j = 0; j < J; ++j) order[at[designs[j].d - 1]++] = static_cast<uint32_t>(j);
+            uint32_t* d_order = nullptr;
+            if ((st = plan_alloc(pl, &d_order, order.size())) != MCD_OK) return st;
+            if ((st = plan_upload(pl, d_order, order)) != MCD_OK) return st;
+            pl->fdims.order = d_order;
+        }
+    }
     if (!pl->rlaunches.empty()) {
         if ((st = plan_alloc(pl, &pl->d_rfams, rt.fams.size())) != MCD_OK) return st;
         if ((st = plan_alloc(pl, &pl->d_rsegs, rt.segs.size())) != MCD_OK) return st;
@@ -883,7 +896,7 @@ mcd_status enqueue(mcd_plan* pl, const LaunchArgs& a, cudaStream_t stream) {
     fp.g_lr = a.g_lr;
     fp.g_sig = a.g_sig;
     fp.g_se = a.g_se;
-    MCD_CUDA(a.grad ? launch_finalize_grad(fp, pl->dims, stream) : launch_finalize(fp, false, stream), "finalize launch");
+    MCD_CUDA(a.grad ? launch_finalize_grad(fp, pl->fdims, stream) : launch_finalize(fp, stream), "finalize launch");
     return MCD_OK;
 }
 

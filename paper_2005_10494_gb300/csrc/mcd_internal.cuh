@@ -120,7 +120,7 @@ struct FinalizeParams {
     double*          g_sig;
     double*          g_se;
 };
-cudaError_t launch_finalize(const FinalizeParams& p, bool grad, cudaStream_t stream);
+cudaError_t launch_finalize(const FinalizeParams& p, cudaStream_t stream);
 
 cudaError_t launch_debug_normals(uint64_t seed, uint64_t key, uint64_t m_begin, uint64_t count,
                                  float* z32, double* z64, uint32_t* words, cudaStream_t stream);
