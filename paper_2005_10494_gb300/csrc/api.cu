@@ -129,6 +129,7 @@ struct mcd_plan {
     bool stream_ordered = false;     // one-shot plan: allocations on a stream
     cudaStream_t alloc_stream = nullptr;
     int32_t S = 0, J = 0, region = 0, k = 0, flags = 0;
+    int32_t max_d = 1;               // largest dimension of a scenario
     bool fp64 = false;
     std::vector<Segment> segs;       // sampling launches, in order
     std::vector<int> seg_of_d;       // segment index of each dimension, -1 if none
@@ -435,6 +436,7 @@ mcd_status plan_build(mcd_ctx* ctx, const mcd_problem* pr, int32_t flags, int32_
 
     std::vector<int64_t> sig_off(S), L_off(S);
     std::vector<int32_t> scen_d(pr->scen_d, pr->scen_d + S);
+    pl->max_d = *std::max_element(scen_d.begin(), scen_d.end());
     int64_t so = 0, lo = 0;
     for (int s = 0; s < S; ++s) {
         sig_off[s] = so;
@@ -794,7 +796,7 @@ mcd_status enqueue(mcd_plan* pl, const LaunchArgs& a, cudaStream_t stream) {
     if (pl->J > 0) MCD_CUDA(cudaMemsetAsync(pl->d_hits, 0, sizeof(unsigned long long) * pl->J, stream), "memset");
     if (a.grad && pl->gacc_len)
         MCD_CUDA(cudaMemsetAsync(pl->d_gacc, 0, sizeof(unsigned long long) * pl->gacc_len, stream), "memset");
-    MCD_CUDA(launch_cholesky(pl->Sigma, pl->d_sig_off, pl->d_scen_d, pl->d_L_off, pl->S, pl->d_L32, pl->d_L64,
+    MCD_CUDA(launch_cholesky(pl->Sigma, pl->d_sig_off, pl->d_scen_d, pl->d_L_off, pl->S, pl->max_d, pl->d_L32, pl->d_L64,
                              pl->d_scen_ok, ctx->d_status, stream), "cholesky launch");
     // under stream capture the timing events must become event-record nodes
     // of the graph (cudaEventRecordExternal), not capture-internal joins

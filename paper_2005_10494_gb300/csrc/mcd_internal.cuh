@@ -96,7 +96,7 @@ int shared_designs_per_thread(int d, bool grad);
 int shared_batch_draws(int d);
 
 cudaError_t launch_cholesky(const double* Sigma, const int64_t* sig_off, const int32_t* scen_d,
-                            const int64_t* L_off, int n_scen, float* L32, double* L64,
+                            const int64_t* L_off, int n_scen, int max_d, float* L32, double* L64,
                             int32_t* scen_ok, DevStatus* status, cudaStream_t stream);
 
 struct FinalizeParams {

@@ -51,7 +51,9 @@ std::mutex g_scratch_mu;
 
 // Sigma = L L^T for the one scenario (FP64, lower triangle read), FP32 copy.
 __global__ void __launch_bounds__(32) noalloc_cholesky_kernel(const double* __restrict__ Sigma, int d, NoAllocScratch* sc) {
-    const bool good = warp_factor(Sigma, d, sc->L64, sc->L32);
+    bool good = false;
+    if (d > kCholThreadD) good = warp_factor(Sigma, d, sc->L64, sc->L32);
+    else if (threadIdx.x == 0) good = thread_factor(Sigma, d, sc->L64, sc->L32);
     if (threadIdx.x == 0) sc->ok = good ? 1 : 0;
 }
 

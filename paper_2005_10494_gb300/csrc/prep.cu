@@ -11,18 +11,19 @@ namespace mcd {
 
 namespace {
 
-// Sigma_s = L L^T, a warp per scenario.
-constexpr int kCholWarps = 2;
-__global__ void __launch_bounds__(32 * kCholWarps) cholesky_kernel(const double* __restrict__ Sigma,
-                                                                   const int64_t* __restrict__ sig_off,
-                                                                   const int32_t* __restrict__ scen_d,
-                                                                   const int64_t* __restrict__ L_off, int n_scen,
-                                                                   float* __restrict__ L32, double* __restrict__ L64,
-                                                                   int32_t* __restrict__ scen_ok, DevStatus* status) {
-    const int s = blockIdx.x * kCholWarps + (threadIdx.x >> 5);
+// Sigma_s = L L^T, a warp or a thread per scenario.
+constexpr int kCholWarps = 2, kCholThreads = 64;
+
+template <bool WARP>
+__global__ void __launch_bounds__(64) cholesky_kernel(const double* __restrict__ Sigma, const int64_t* __restrict__ sig_off,
+                                                      const int32_t* __restrict__ scen_d, const int64_t* __restrict__ L_off,
+                                                      int n_scen, float* __restrict__ L32, double* __restrict__ L64,
+                                                      int32_t* __restrict__ scen_ok, DevStatus* status) {
+    const int s = WARP ? blockIdx.x * kCholWarps + (threadIdx.x >> 5) : blockIdx.x * kCholThreads + threadIdx.x;
     if (s >= n_scen) return;
-    const bool good = warp_factor(Sigma + sig_off[s], scen_d[s], L64 + L_off[s], L32 + L_off[s]);
-    if ((threadIdx.x & 31) == 0) {
+    const bool good = WARP ? warp_factor(Sigma + sig_off[s], scen_d[s], L64 + L_off[s], L32 + L_off[s])
+                           : thread_factor(Sigma + sig_off[s], scen_d[s], L64 + L_off[s], L32 + L_off[s]);
+    if (!WARP || (threadIdx.x & 31) == 0) {
         scen_ok[s] = good ? 1 : 0;
         if (!good) set_status(status, MCD_ENOTSPD, s);
     }
@@ -59,11 +60,20 @@ __global__ void debug_normals_kernel(uint64_t seed, uint64_t key, uint64_t m_beg
 
 }  // namespace
 
+// A warp per scenario costs 32 lanes' worth of the FP64 rate: us for a thread and
+// for a warp each, with 1024, 2048, 4096 and 8192 scenarios: d = 6 16.5, 18.5; 16.4,
+// 29; 16.5, 55; 16.5, 103; d = 10 41, 29; 41, 45; 41, 90; 41, 172; d = 20 190, 57; 194, 96; 195,
+// 191; 197, 373.  `max_d` is the largest dimension of the scenarios, whose chain a
+// launch of threads waits for.
 cudaError_t launch_cholesky(const double* Sigma, const int64_t* sig_off, const int32_t* scen_d,
-                            const int64_t* L_off, int n_scen, float* L32, double* L64,
+                            const int64_t* L_off, int n_scen, int max_d, float* L32, double* L64,
                             int32_t* scen_ok, DevStatus* status, cudaStream_t stream) {
-    cholesky_kernel<<<(n_scen + kCholWarps - 1) / kCholWarps, 32 * kCholWarps, 0, stream>>>(
-        Sigma, sig_off, scen_d, L_off, n_scen, L32, L64, scen_ok, status);
+    if (max_d > kCholThreadD && n_scen <= 230 * (max_d - 4))
+        cholesky_kernel<true><<<(n_scen + kCholWarps - 1) / kCholWarps, 32 * kCholWarps, 0, stream>>>(
+            Sigma, sig_off, scen_d, L_off, n_scen, L32, L64, scen_ok, status);
+    else
+        cholesky_kernel<false><<<(n_scen + kCholThreads - 1) / kCholThreads, kCholThreads, 0, stream>>>(
+            Sigma, sig_off, scen_d, L_off, n_scen, L32, L64, scen_ok, status);
     return cudaGetLastError();
 }
 
