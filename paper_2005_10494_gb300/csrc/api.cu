@@ -78,16 +78,56 @@ struct RankLaunch {
     int64_t n_tiles = 0, n_units = 0;
 };
 
-// The ranked path queues three kernels and builds rows per chunk, about 20 us
-// together; the kernel that tests every design against every draw spends its
-// threads in rounds of 256 designs.  Measured on one group (forward, d = 1, 3,
-// 5, 10, 20, 32..2048 designs, 1e4..6.4e5 draws) the two cross where
-// d x draws x ceil(designs / 256) is about 1.25e6: at d = 3, 32 x 640k takes
-// 69 us there and 59 us ranked, 512 x 160k 51 and 60 us; at d = 20, 32 x 160k
-// 255 and 223 us.  The work of a dimension's groups adds up (one launch), and
-// groups of few draws do not pay for their rows.
-constexpr double kRankMinWork = 1.25e6;
-constexpr uint64_t kRankMinDraws = 16384;
+// When the ranked path pays: time in us of a dimension's common-random-number
+// groups in either path.  The shared-draw kernel makes its draws once per chunk
+// and tests them in rounds of 256 designs; the ranked path makes them once per
+// family, or-s words of 32 designs, builds rows per chunk and sorts.  The
+// coefficients are a least-squares fit (90 % of the cases within 25 %) to 420 forward
+// plans of d = 1..20, 1..400 groups, 32..6000 designs and 8e3..1.5e6 draws in both
+// paths.  Predicted 15 % ahead, the ranked path was no more than 2 % slower in any
+// of them: one group of d = 3, 32 x 1e6 takes 89 us there and 66 ranked, 4096 x 50k
+// 75 and 81; d = 1, 32 groups of 700 x 16k 58 and 84; d = 10, 4096 x 16k 106 and 94.
+// A line through d x draws x rounds (1.25e6) left calls of 50 to 90 us up to 30 %
+// slower than they had been.
+constexpr double kRankMargin = 1.15;
+constexpr uint64_t kRankMinDraws = 16384;       // groups of few draws do not pay for their rows
+
+class RankCost {
+public:
+    void add(int d, size_t designs, uint64_t draws) {
+        const double n = 1e-6 * static_cast<double>(draws);
+        const size_t cap = static_cast<size_t>(kSharedThreads) * shared_designs_per_thread(d, false);
+        const size_t nch = (designs + cap - 1) / cap, per = (designs + nch - 1) / nch;
+        const double rounds = static_cast<double>((per + kSharedThreads - 1) / kSharedThreads);
+        direct_ += static_cast<double>(nch) * n * (1.25 * d * d + 13.7 * rounds * d);
+        const size_t fam = static_cast<size_t>(rank_family(d));
+        for (size_t c = 0; c < designs; c += fam) {
+            const int cnt = static_cast<int>(std::min(fam, designs - c)), w = rank_words(d, cnt);
+            const double chunks = (cnt + 32 * w - 1) / (32 * w);
+            const double rows = ((d + 32 / w - 1) / (32 / w)) * (32.0 * w + 1.0) / 256.0;   // of one chunk
+            ranked_ += n * (1.82 * d + 0.353 * d * d + 0.319 * d * w * chunks);
+            rows_ += rows * chunks;
+            most_rows_ = std::max(most_rows_, rows);
+            sorts_ += d;
+            most_keys_ = std::max(most_keys_, cnt);
+            classes_ |= w;
+        }
+    }
+    bool ranked(int sms) const {
+        int keys = 32;
+        while (keys < most_keys_) keys <<= 1;
+        const int further = (classes_ & (classes_ - 1)) == 0 ? 0 : classes_ == 28 ? 2 : 1;   // words 4, 8, 16
+        const double t = 57.7 + ranked_ + 4.31 * std::max(most_rows_, rows_ / sms) +
+                         13.1 * static_cast<double>((sorts_ + sms - 1) / sms) * keys / kRankMaxFamily +
+                         25.0 * further;                 // three more launches for each further class of families
+        return t * kRankMargin < 37.6 + direct_;
+    }
+
+private:
+    double direct_ = 0.0, ranked_ = 0.0, rows_ = 0.0, most_rows_ = 0.0;
+    int64_t sorts_ = 0;
+    int most_keys_ = 0, classes_ = 0;
+};
 
 // Blocks per SM for which the tiles of shared draws of a gradient plan are sized.
 // They fix which draws are summed in FP32 before the fixed-point sums, and which
@@ -418,18 +458,15 @@ mcd_status plan_build(mcd_ctx* ctx, const mcd_problem* pr, int32_t flags, int32_
             if (pr->n_draws[j] == 0) continue;
             by[std::make_tuple(pr->design_scen[j], pr->key[j], begin, pr->n_draws[j])].push_back(j);
         }
-        std::vector<double> rank_work(MCD_MAX_D + 1, 0.0);
-        for (auto& kv : by) {
-            const uint64_t n = std::get<3>(kv.first);
-            const int d = pr->scen_d[std::get<0>(kv.first)];
-            if (static_cast<int>(kv.second.size()) >= MCD_SHARED_MIN && n >= kRankMinDraws)
-                rank_work[d] += static_cast<double>(d) * static_cast<double>(n) * static_cast<double>((kv.second.size() + 255) / 256);
-        }
+        std::vector<RankCost> cost(MCD_MAX_D + 1);
+        for (auto& kv : by)
+            if (static_cast<int>(kv.second.size()) >= MCD_SHARED_MIN && std::get<3>(kv.first) >= kRankMinDraws)
+                cost[pr->scen_d[std::get<0>(kv.first)]].add(pr->scen_d[std::get<0>(kv.first)], kv.second.size(), std::get<3>(kv.first));
         for (auto& kv : by) {
             if (static_cast<int>(kv.second.size()) < MCD_SHARED_MIN) continue;
             for (int j : kv.second) is_shared[j] = 1;
             const bool ranked = !grad_kernel && std::get<3>(kv.first) >= kRankMinDraws &&
-                                rank_work[pr->scen_d[std::get<0>(kv.first)]] >= kRankMinWork;
+                                cost[pr->scen_d[std::get<0>(kv.first)]].ranked(ctx->sm_count);
             (ranked ? rgroups : groups).push_back(std::move(kv.second));
         }
     }

@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 
 # designs, draws: 512 and 4096 thresholds per coordinate, which take 12 and 98 KB
 # of shared memory in one kernel and as many more words in the other
-D, SMALL, LARGE = 6, (300, 300_000), (4096, 30_000)
+D, SMALL, LARGE = 6, (300, 400_000), (4096, 70_000)
 
 
 def grid(designs, draws, seed):
