@@ -67,6 +67,7 @@ struct SharedSeg {
     int64_t tile_draws = 0;
     int grid = 0;
     int blocks_per_sm = 0;
+    bool boxed = false;              // gradient plans: the adjoint launch takes box_kernel
 };
 
 // One round of the ranked shared-draw path: families [fam0, fam0 + n_fam) of
@@ -133,6 +134,18 @@ private:
 // They fix which draws are summed in FP32 before the fixed-point sums, and which
 // share a batch slot, so results do not move with a kernel's register count.
 constexpr int kTileBlocks[MCD_MAX_D + 1] = {0, 4, 3, 3, 2, 2, 2, 2, 2, 2, 2, 2, 2, 1, 2, 1, 2, 1, 2, 1, 2};
+// Where box_kernel (boxed.cuh) is the faster adjoint: it sets the boxes up per tile and
+// takes the draws that are left one at a time, which costs more than it saves where
+// a launch waits on latency.  Time of the direct over the boxed kernel's on grids of
+// 36 to 4096 designs and 1e3 to 2e6 draws (geometric mean; least, most): d = 10, tiles of
+// one batch 0.97 (0.90, 1.07), of more 1.07 (1.00, 1.12); d = 11, no more tiles than
+// resident blocks 0.96 (0.92, 0.97), more 1.06 (0.91, 1.30); d = 12, more 1.05 (0.95, 1.26);
+// d = 17, 18, 19 and 20 at all sizes 1.05 (0.94, 1.16), 1.06 (0.97, 1.23), 1.08 (0.95, 1.24)
+// and 1.11 (0.97, 1.48).
+bool box_pays(int d, int64_t tiles, int64_t batches, int64_t resident) {
+    return d == 10 ? batches >= 2 : d == 11 || d == 12 ? tiles > resident : d >= 17;
+}
+
 constexpr size_t kRankWorkspace = 64ull << 20;   // ranks of one round: well inside the 129 MB L2
 constexpr int kRankFamilies = 256;               // families of one round (their thresholds: 74 KB each at d=3)
 
@@ -562,7 +575,7 @@ mcd_status plan_build(mcd_ctx* ctx, const mcd_problem* pr, int32_t flags, int32_
             SharedSeg sg;
             sg.d = d;
             int bps = 0;
-            cudaError_t e = shared_occupancy(d, grad_kernel, &bps);
+            cudaError_t e = shared_occupancy(d, grad_kernel, false, &bps);
             if (e != cudaSuccess) return cuda_fail(ctx, e, "occupancy query");
             sg.blocks_per_sm = std::max(1, bps);
             const double bd = shared_batch_draws(d);
@@ -687,6 +700,14 @@ mcd_status plan_build(mcd_ctx* ctx, const mcd_problem* pr, int32_t flags, int32_
             sg.tile_begin = pos;
             while (pos < static_cast<int64_t>(stiles.size()) && scen_d[stiles[pos].scen] == sg.d) ++pos;
             sg.n_tiles = pos - sg.tile_begin;
+            sg.boxed = grad_kernel && box_pays(sg.d, sg.n_tiles, sg.tile_draws / shared_batch_draws(sg.d),
+                                               static_cast<int64_t>(kTileBlocks[sg.d]) * ctx->sm_count);
+            if (sg.boxed) {
+                int bps = 0;
+                cudaError_t e = shared_occupancy(sg.d, true, true, &bps);
+                if (e != cudaSuccess) return cuda_fail(ctx, e, "occupancy query");
+                sg.blocks_per_sm = std::max(1, bps);
+            }
             const int64_t g = static_cast<int64_t>(sg.blocks_per_sm) * ctx->sm_count;
             sg.grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(g, sg.n_tiles)));
         }
@@ -866,7 +887,7 @@ mcd_status enqueue(mcd_plan* pl, const LaunchArgs& a, cudaStream_t stream) {
         base_params(sp);
         sp.n_tiles = sg.n_tiles;
         sp.ticket = pl->d_ticket + pl->segs.size() + q;
-        MCD_CUDA(launch_shared(sg.d, a.grad, sp, pl->d_stiles + sg.tile_begin, pl->d_slist, sg.grid, stream),
+        MCD_CUDA(launch_shared(sg.d, a.grad, sg.boxed, sp, pl->d_stiles + sg.tile_begin, pl->d_slist, sg.grid, stream),
                  "shared-draw launch");
     }
     for (const RankLaunch& l : pl->rlaunches) {

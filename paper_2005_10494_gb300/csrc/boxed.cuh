@@ -1,4 +1,4 @@
-// Shared-draw adjoint at d >= 9 (kBoxed): draws that no design of a warp can tell
+// Shared-draw adjoint at d = 10..12 and 17..20 (kBoxed): draws that no design of a warp can tell
 // apart are added, or dropped, without testing them design by design.
 #pragma once
 
@@ -6,19 +6,17 @@
 
 namespace mcd {
 
-// Where the box pays: from d = 9 on, where a thread has one design and a pair
-// costs 50 to 105 instructions, bound by issue and the row loads.  Ms of the
-// sampling kernel, without and with it, on 64 x 64 grids of wide range (2e5
-// draws): d = 9 1.37, 1.28; 10 1.77, 1.64; 12 1.80, 1.53; 20 3.73, 3.49; where a
-// word spans little of a threshold's range it saves more (d = 20, 4096 designs,
-// whole step 12.5, 8.0).  At d = 13 and 15 one block fits an SM and the shorter
-// loops leave latencies open: 2.76, 3.04 and 3.35, 3.77.  At d = 5..8, two
-// designs per thread, 0.72, 0.87 and 1.70, 1.96.
-// Thresholds in no order (1500 random designs) fall back to the direct loop, within
-// 1 % at d <= 12, 17 and 19; at even d from 14 on a few more of its registers
-// spill: 2 to 5 % slower, the price of the 3 to 36 % on grids.
+// The dimensions that have the kernel.  Time without it / with it on 32 x 32, 64 x 64
+// and 9 x 15 grids of 1 to 12 ms (geometric mean, least), and on as many scattered
+// designs, which fall back to the direct loop: d = 9 0.97, 0.90 and 0.99; 10 1.07, 1.00
+// and 0.99; 11 1.15, 1.00 and 1.00; 12 1.16, 1.00 and 0.99; 14 1.04, 0.96 and 0.98; 16 1.07,
+// 0.96 and 0.95; 17 1.09, 1.00 and 1.00; 18 1.12, 1.01 and 0.98; 19 1.13, 1.02 and 1.00; 20
+// 1.24, 1.03 and 0.98.  At d = 13 and 15 one block fits an SM and the shorter loops
+// leave latencies open: 0.91, 0.89.  At d = 5..8, two designs per thread, 0.83, 0.87.
+// Not where it loses on either (9, 14, 16); at 18 and 20 scattered designs are up to
+// 3.6 % slower in the sampling, the price of 12 and 24 % on grids.
 template <int D>
-constexpr bool kBoxed = D >= 9 && D != 13 && D != 15;
+constexpr bool kBoxed = (D >= 10 && D <= 12) || D >= 17;
 
 // Whole numbers in the order of the floats: a warp's extremes take one reduction
 // instead of ten shuffles and minima (0.5 to 1 % where a tile has 256 draws).
@@ -284,17 +282,17 @@ __device__ __forceinline__ void box_body(const SampleParams& P, const SharedTile
     }
 }
 
-// Three resident blocks per SM at d <= 3, two up to d = 12 and at even d, one at
-// the odd d above, whose batches take more than half of the shared memory.
+// Two resident blocks per SM, one at odd d from 17 on, whose batches take more than
+// half of the shared memory.
 template <int D>
-__global__ void __launch_bounds__(kSharedThreads, D <= 3 ? 3 : D <= 12 || D % 2 == 0 ? 2 : 1)
+__global__ void __launch_bounds__(kSharedThreads, D <= 12 || D % 2 == 0 ? 2 : 1)
 box_kernel(const __grid_constant__ SampleParams P, const SharedTile* __restrict__ tiles,
            const uint32_t* __restrict__ list) {
     box_body<D>(P, tiles, list);
 }
 
 template <int D>
-const void* adjoint_fn() {
+const void* box_fn() {
     if constexpr (kBoxed<D>) return reinterpret_cast<const void*>(&box_kernel<D>);
     else return shared_fn<D, true>();
 }

@@ -88,10 +88,11 @@ cudaError_t launch_sample(int d_lo, int d_hi, bool grad, bool fp64, const Sample
 int  sample_kernel_regs(int d_lo, int d_hi, bool grad, bool fp64);
 cudaError_t sample_occupancy(int d_lo, int d_hi, bool grad, bool fp64, int threads, int* blocks);
 
-// Shared-draw kernel of dimension d (FP32 only).
-cudaError_t launch_shared(int d, bool grad, const SampleParams& p, const SharedTile* tiles, const uint32_t* list,
-                          int grid, cudaStream_t stream);
-cudaError_t shared_occupancy(int d, bool grad, int* blocks);
+// Shared-draw kernel of dimension d (FP32 only); `boxed`: the adjoint's box_kernel
+// where the dimension has one, the same results.
+cudaError_t launch_shared(int d, bool grad, bool boxed, const SampleParams& p, const SharedTile* tiles,
+                          const uint32_t* list, int grid, cudaStream_t stream);
+cudaError_t shared_occupancy(int d, bool grad, bool boxed, int* blocks);
 int shared_designs_per_thread(int d, bool grad);
 int shared_batch_draws(int d);
 

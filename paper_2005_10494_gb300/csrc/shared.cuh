@@ -330,6 +330,9 @@ __device__ __forceinline__ void shared_body(const SampleParams& P, const SharedT
                 t[q][i] = dsg[q] >= 0 ? static_cast<float>(tt) : INFINITY;
             }
         }
+        // a warp without designs only makes its share of the draws (100 groups of 33
+        // designs x 16k draws: d = 9 695 -> 533 us, d = 16 1614 -> 1328 us)
+        const bool mine = !(GRAD && DPT == 1) || __any_sync(0xffffffffu, dsg[0] >= 0);
         __syncthreads();                              // sL complete
         if (!ok) continue;                            // block-uniform; the next ticket read is behind a barrier
 
@@ -371,7 +374,8 @@ __device__ __forceinline__ void shared_body(const SampleParams& P, const SharedT
             const int nb = static_cast<int>(min(static_cast<uint32_t>(SS::kBD), (ngroups - g0) * S::kG));
             // nq is block-uniform: one branch per batch picks the loop for
             // exactly nq designs per thread
-            if (nq >= DPT) test_draws<D, GRAD, DPT, DPT>(sy, sz, nb, t, nhl2e, wsk, cnt, A, G);
+            if (!mine) {}
+            else if (nq >= DPT) test_draws<D, GRAD, DPT, DPT>(sy, sz, nb, t, nhl2e, wsk, cnt, A, G);
             else if constexpr (DPT > 1) {
                 if (nq == 1) test_draws<D, GRAD, DPT, 1>(sy, sz, nb, t, nhl2e, wsk, cnt, A, G);
                 else if constexpr (DPT > 2) {
