@@ -82,15 +82,17 @@ struct RankLaunch {
 // When the ranked path pays: time in us of a dimension's common-random-number
 // groups in either path.  The shared-draw kernel makes its draws once per chunk
 // and tests them in rounds of 256 designs; the ranked path makes them once per
-// family, or-s words of 32 designs, builds rows per chunk and sorts.  The
-// coefficients are a least-squares fit (90 % of the cases within 25 %) to 420 forward
-// plans of d = 1..20, 1..400 groups, 32..6000 designs and 8e3..1.5e6 draws in both
-// paths.  Predicted 15 % ahead, the ranked path was no more than 2 % slower in any
-// of them: one group of d = 3, 32 x 1e6 takes 89 us there and 66 ranked, 4096 x 50k
-// 75 and 81; d = 1, 32 groups of 700 x 16k 58 and 84; d = 10, 4096 x 16k 106 and 94.
-// A line through d x draws x rounds (1.25e6) left calls of 50 to 90 us up to 30 %
-// slower than they had been.
+// family, or-s words of 32 designs, builds rows per chunk, sorts, and runs its three
+// kernels once for every 256 families.  The coefficients are a least-squares fit
+// (90 % of the cases within 35 %) to 668 forward plans of d = 1..20, 1..1500 groups,
+// 32..6000 designs and 12e3..1.5e6 draws in both paths.  Predicted 15 % ahead, the
+// ranked path was slower in one of them (d = 5, 32 groups of 100 x 16k: 90, 100): one
+// group of d = 3, 32 x 1e6 takes 89 us there and 66 ranked, 4096 x 50k 75 and 81; d = 1,
+// 32 groups of 700 x 16k 58 and 84, 300 of 100 x 16k 165 and 188; d = 10, 4096 x 16k 106 and
+// 94.  A line through d x draws x rounds (1.25e6) left calls of 50 to 190 us up to
+// 30 % slower than they had been.
 constexpr double kRankMargin = 1.15;
+constexpr int kRankFamilies = 256;              // families of one round (their thresholds: 74 KB each at d=3)
 constexpr uint64_t kRankMinDraws = 16384;       // groups of few draws do not pay for their rows
 
 class RankCost {
@@ -100,16 +102,17 @@ public:
         const size_t cap = static_cast<size_t>(kSharedThreads) * shared_designs_per_thread(d, false);
         const size_t nch = (designs + cap - 1) / cap, per = (designs + nch - 1) / nch;
         const double rounds = static_cast<double>((per + kSharedThreads - 1) / kSharedThreads);
-        direct_ += static_cast<double>(nch) * n * (1.25 * d * d + 13.7 * rounds * d);
+        direct_ += static_cast<double>(nch) * n * (6.4 + 0.843 * d * d + 13.6 * rounds * d);
         const size_t fam = static_cast<size_t>(rank_family(d));
         for (size_t c = 0; c < designs; c += fam) {
             const int cnt = static_cast<int>(std::min(fam, designs - c)), w = rank_words(d, cnt);
             const double chunks = (cnt + 32 * w - 1) / (32 * w);
             const double rows = ((d + 32 / w - 1) / (32 / w)) * (32.0 * w + 1.0) / 256.0;   // of one chunk
-            ranked_ += n * (1.82 * d + 0.353 * d * d + 0.319 * d * w * chunks);
+            ranked_ += n * (2.73 + 2.31 * d + 0.204 * d * d + 0.26 * d * w * chunks);
             rows_ += rows * chunks;
             most_rows_ = std::max(most_rows_, rows);
             sorts_ += d;
+            ++families_;
             most_keys_ = std::max(most_keys_, cnt);
             classes_ |= w;
         }
@@ -118,15 +121,16 @@ public:
         int keys = 32;
         while (keys < most_keys_) keys <<= 1;
         const int further = (classes_ & (classes_ - 1)) == 0 ? 0 : classes_ == 28 ? 2 : 1;   // words 4, 8, 16
-        const double t = 57.7 + ranked_ + 4.31 * std::max(most_rows_, rows_ / sms) +
-                         13.1 * static_cast<double>((sorts_ + sms - 1) / sms) * keys / kRankMaxFamily +
+        const double t = 56.0 + ranked_ + 5.46 * std::max(most_rows_, rows_ / sms) +
+                         11.8 * static_cast<double>((sorts_ + sms - 1) / sms) * keys / kRankMaxFamily +
+                         95.3 * static_cast<double>((families_ - 1) / kRankFamilies) +
                          25.0 * further;                 // three more launches for each further class of families
-        return t * kRankMargin < 37.6 + direct_;
+        return t * kRankMargin < 38.5 + direct_;
     }
 
 private:
     double direct_ = 0.0, ranked_ = 0.0, rows_ = 0.0, most_rows_ = 0.0;
-    int64_t sorts_ = 0;
+    int64_t sorts_ = 0, families_ = 0;
     int most_keys_ = 0, classes_ = 0;
 };
 
@@ -147,7 +151,6 @@ bool box_pays(int d, int64_t tiles, int64_t batches, int64_t resident) {
 }
 
 constexpr size_t kRankWorkspace = 64ull << 20;   // ranks of one round: well inside the 129 MB L2
-constexpr int kRankFamilies = 256;               // families of one round (their thresholds: 74 KB each at d=3)
 
 // Which tiles a plan keeps (the autotuner times filtered plans).
 struct TileFilter {
