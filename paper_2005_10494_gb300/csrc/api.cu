@@ -769,18 +769,33 @@ mcd_status plan_build(mcd_ctx* ctx, const mcd_problem* pr, int32_t flags, int32_
         }
     }
     if (!pl->rlaunches.empty()) {
-        if ((st = plan_alloc(pl, &pl->d_rfams, rt.fams.size())) != MCD_OK) return st;
-        if ((st = plan_alloc(pl, &pl->d_rsegs, rt.segs.size())) != MCD_OK) return st;
-        if ((st = plan_alloc(pl, &pl->d_ritems, rt.items.size())) != MCD_OK) return st;
-        if ((st = plan_alloc(pl, &pl->d_rlist, rt.list.size())) != MCD_OK) return st;
-        if ((st = plan_alloc(pl, &pl->d_rdistinct, rt.thresholds)) != MCD_OK) return st;
-        if ((st = plan_alloc(pl, &pl->d_rpos, rt.thresholds)) != MCD_OK) return st;
-        if ((st = plan_alloc(pl, &pl->d_rndistinct, rt.coords)) != MCD_OK) return st;
-        if ((st = plan_alloc(pl, &pl->d_ranks, rt.ws_bytes / sizeof(uint16_t))) != MCD_OK) return st;
-        if ((st = plan_upload(pl, pl->d_rfams, rt.fams)) != MCD_OK) return st;
-        if ((st = plan_upload(pl, pl->d_rsegs, rt.segs)) != MCD_OK) return st;
-        if ((st = plan_upload(pl, pl->d_ritems, rt.items)) != MCD_OK) return st;
-        if ((st = plan_upload(pl, pl->d_rlist, rt.list)) != MCD_OK) return st;
+        // one block, the tables first: one allocation and one copy
+        size_t at = 0;
+        auto place = [&](size_t bytes) {
+            const size_t here = at;
+            at = (at + bytes + 255) / 256 * 256;
+            return here;
+        };
+        const size_t fams = place(rt.fams.size() * sizeof(RankFam)), segs = place(rt.segs.size() * sizeof(RankSeg));
+        const size_t items = place(rt.items.size() * sizeof(RankItem)), lists = place(rt.list.size() * sizeof(uint32_t));
+        std::vector<unsigned char> tables(at);
+        std::memcpy(tables.data() + fams, rt.fams.data(), rt.fams.size() * sizeof(RankFam));
+        std::memcpy(tables.data() + segs, rt.segs.data(), rt.segs.size() * sizeof(RankSeg));
+        std::memcpy(tables.data() + items, rt.items.data(), rt.items.size() * sizeof(RankItem));
+        std::memcpy(tables.data() + lists, rt.list.data(), rt.list.size() * sizeof(uint32_t));
+        const size_t distinct = place(rt.thresholds * sizeof(float)), pos = place(rt.thresholds * sizeof(uint16_t));
+        const size_t ndistinct = place(rt.coords * sizeof(int32_t)), ranks = place(rt.ws_bytes);
+        unsigned char* block = nullptr;
+        if ((st = plan_alloc(pl, &block, at)) != MCD_OK) return st;
+        if ((st = plan_upload(pl, block, tables)) != MCD_OK) return st;
+        pl->d_rfams = reinterpret_cast<RankFam*>(block + fams);
+        pl->d_rsegs = reinterpret_cast<RankSeg*>(block + segs);
+        pl->d_ritems = reinterpret_cast<RankItem*>(block + items);
+        pl->d_rlist = reinterpret_cast<uint32_t*>(block + lists);
+        pl->d_rdistinct = reinterpret_cast<float*>(block + distinct);
+        pl->d_rpos = reinterpret_cast<uint16_t*>(block + pos);
+        pl->d_rndistinct = reinterpret_cast<int32_t*>(block + ndistinct);
+        pl->d_ranks = reinterpret_cast<uint16_t*>(block + ranks);
     }
 
     if ((st = plan_upload(pl, pl->d_designs, designs)) != MCD_OK) return st;
