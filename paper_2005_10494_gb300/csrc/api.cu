@@ -144,7 +144,7 @@ constexpr int kTileBlocks[MCD_MAX_D + 1] = {0, 4, 3, 3, 2, 2, 2, 2, 2, 2, 2, 2, 
 // 36 to 4096 designs and 1e3 to 2e6 draws (geometric mean; least, most): d = 10, tiles of
 // one batch 0.97 (0.90, 1.07), of more 1.07 (1.00, 1.12); d = 11, no more tiles than
 // resident blocks 0.96 (0.92, 0.97), more 1.06 (0.91, 1.30); d = 12, more 1.05 (0.95, 1.26);
-// d = 17, 18, 19 and 20 at all sizes 1.05 (0.94, 1.16), 1.06 (0.97, 1.23), 1.08 (0.95, 1.24)
+// d = 17, 18, 19 and 20 at all sizes 1.05 (0.94, 1.16), 1.10 (0.98, 1.36), 1.08 (0.95, 1.24)
 // and 1.11 (0.97, 1.48).
 bool box_pays(int d, int64_t tiles, int64_t batches, int64_t resident) {
     return d == 10 ? batches >= 2 : d == 11 || d == 12 ? tiles > resident : d >= 17;

@@ -10,11 +10,11 @@ namespace mcd {
 // and 9 x 15 grids of 1 to 12 ms (geometric mean, least), and on as many scattered
 // designs, which fall back to the direct loop: d = 9 0.97, 0.90 and 0.99; 10 1.07, 1.00
 // and 0.99; 11 1.15, 1.00 and 1.00; 12 1.16, 1.00 and 0.99; 14 1.04, 0.96 and 0.98; 16 1.07,
-// 0.96 and 0.95; 17 1.09, 1.00 and 1.00; 18 1.12, 1.01 and 0.98; 19 1.13, 1.02 and 1.00; 20
-// 1.24, 1.03 and 0.98.  At d = 13 and 15 one block fits an SM and the shorter loops
+// 0.96 and 0.95; 17 1.09, 1.00 and 1.00; 18 1.12, 1.01 and 0.98 (before
+// kAgain, below); 19 1.13, 1.02 and 1.00; 20 1.24, 1.03 and 0.97.  At d = 13 and 15 one block fits an SM and the shorter loops
 // leave latencies open: 0.91, 0.89.  At d = 5..8, two designs per thread, 0.83, 0.87.
-// Not where it loses on either (9, 14, 16); at 18 and 20 scattered designs are up to
-// 3.6 % slower in the sampling, the price of 12 and 24 % on grids.
+// Not where it loses on either (9, 14, 16); at 20 scattered designs are 2 to 4 % slower
+// in the sampling, the price of 24 % on grids.
 template <int D>
 constexpr bool kBoxed = (D >= 10 && D <= 12) || D >= 17;
 
@@ -75,6 +75,11 @@ __device__ __forceinline__ void box_draws(const float* sy, const float* sz, int 
     constexpr int DP = SharedShape<D, true>::kDP;
     constexpr int DA = SharedShape<D, true>::kDA;
     static_assert(DPT == 1, "one design per thread");
+    // At d = 18 the differences are formed again where the sigmoid needs them: kept,
+    // they cost 172 bytes of spills more than the direct kernel has (grids 1.06 -> 1.10
+    // of its speed, scattered designs 0.975 -> 0.99).  At d = 10..12, 17, 19 and 20 keeping them
+    // measured 1 to 3 % faster on grids.
+    constexpr bool kAgain = D == 18;
     const float w = fmaxf(wsk, 0.0f);
     for (int d0 = 0; d0 < nb; d0 += 32) {             // rows up to kBD exist: past nb they hold y = -inf
         uint32_t ev[DPT], in[DPT];
@@ -108,13 +113,17 @@ __device__ __forceinline__ void box_draws(const float* sy, const float* sz, int 
                 float dif[D], dmin = 0.0f;
                 const bool test = ev[q] >> b & 1u;      // warp-uniform
                 if (test) {
-                    float y[DP];
+                    float y[DP], v[D];
                     load_row<DP>(sy + (d0 + b) * DP, y);
-                    diffs<D>(t[q], y, dif);
-                    dmin = dif[0];
+                    diffs<D>(t[q], y, v);
+                    dmin = v[0];
 #pragma unroll
-                    for (int i = 1; i < D; i += 2) dmin = i + 1 < D ? fmin3(dmin, dif[i], dif[i + 1]) : fminf(dmin, dif[i]);
+                    for (int i = 1; i < D; i += 2) dmin = i + 1 < D ? fmin3(dmin, v[i], v[i + 1]) : fminf(dmin, v[i]);
                     hit = dmin < 0.0f;
+                    if constexpr (!kAgain) {
+#pragma unroll
+                        for (int i = 0; i < D; ++i) dif[i] = v[i];
+                    }
                 }
                 if constexpr (!SharedShape<D, true>::kCnt) cnt[q] += hit ? 1u : 0u;
                 if (hit) {
@@ -127,6 +136,11 @@ __device__ __forceinline__ void box_draws(const float* sy, const float* sz, int 
                     if constexpr (DA % 2 != 0) A[q][DA - 1] = __fadd_rn(A[q][DA - 1], zz[DA - 1]);
                 }
                 if (test && __any_sync(0xffffffffu, fabsf(dmin) < wsk)) {
+                    if constexpr (kAgain) {
+                        float y[DP];
+                        load_row<DP>(sy + (d0 + b) * DP, y);
+                        diffs<D>(t[q], y, dif);
+                    }
                     float keep[D], prod = 1.0f;
                     const float2 nh2 = make_float2(nhl2e, nhl2e), one2 = make_float2(1.0f, 1.0f);
 #pragma unroll
