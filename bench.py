@@ -289,7 +289,7 @@ def parse_args():
     ap.add_argument("--no-extras", action="store_true", help="skip the d=10/20, smoothing and C3 lines")
     ap.add_argument("--cpu-seconds", type=float, default=12.0, help="target CPU time of the oracle baseline")
     ap.add_argument("--case", default=None, choices=["c2-small", "c4-small", "c5-small", "smooth", "smooth-f32",
-                                                      "c2-shared", "c2-shared-full", "tps", "shared-dims",
+                                                      "c2-shared", "c2-shared-full", "c5-shared", "tps", "shared-dims",
                                                       "perdesign-dims", "tps-timing"],
                     help="run a small profiling case (a few launches, no timing), or one of the timing sweeps "
                          "(shared-dims, perdesign-dims, tps-timing: JSON lines), and exit")
@@ -942,11 +942,18 @@ def paper_problem(pkg, ctx, n_alpha=2000, N1=10240, N2=20480):
             "paper_context": "mean 31.6 s per problem for the whole optimisation on a V100 (Sec. 3; 4.5 h / 513 problems)"}
 
 
+RANKED_THREADS = 512                     # block size of the ranked kernels (the direct shared-draw kernel: 256)
+BOXED_DIMS = (10, 11, 12, 17, 18, 19, 20)   # dimensions whose large adjoint launches take box_kernel
+
+
 def shared_line(pkg, ctx, prob, d, rates, sm_count, h=0.01):
     """A grid whose designs share one stream per scenario (common random
-    numbers) evaluated by the shared-draw kernel, forward and forward +
-    adjoint, against the per-design kernel on the same seed (hits must
-    agree); each with its min-over-pipes bound and FP32-pipe fraction."""
+    numbers), forward and forward + adjoint, against the per-design kernel on
+    the same seed (hits must agree), with the kernels that the plan takes:
+    "direct" tests every design against every draw, and has its min-over-pipes
+    bound and FP32-pipe fraction; "ranked" (large forward groups) and "boxed"
+    (adjoint at BOXED_DIMS) skip most of those tests, so the bound of testing
+    every pair does not hold for them and none is given."""
     import torch
     dp = pkg.DeviceProblem.from_workload(prob)
     jac = torch.as_tensor(prob.jac_packed(), dtype=torch.float64, device="cuda")
@@ -964,12 +971,14 @@ def shared_line(pkg, ctx, prob, d, rates, sm_count, h=0.01):
         ms = plan.kernel_ms()
         same = bool(torch.equal(out["hits"], ref_hits))
         rate = prob.total_draws() / (ms / 1e3)
-        pb = shared_pipe_bound(rates, d, grad, shared_dpt(d, grad), active, sm_count)
-        res["adj" if grad else "fwd"] = {"kernel_ms": ms, "draw_evals_per_s": rate,
-                                         "hits_equal_per_design_kernel": same,
-                                         "pipe_bound": {"binding": pb["binding"], "bound": pb["bound_draw_evals_per_s"],
-                                                        "frac": rate / pb["bound_draw_evals_per_s"]},
-                                         "fp32_pipe_frac": rate * shared_fp32_flops(d, grad, active) / fp32_peak}
+        kernel = "ranked" if plan.config(d)["threads"] == RANKED_THREADS else "boxed" if grad and d in BOXED_DIMS else "direct"
+        line = {"kernel": kernel, "kernel_ms": ms, "draw_evals_per_s": rate, "hits_equal_per_design_kernel": same}
+        if kernel == "direct":
+            pb = shared_pipe_bound(rates, d, grad, shared_dpt(d, grad), active, sm_count)
+            line["pipe_bound"] = {"binding": pb["binding"], "bound": pb["bound_draw_evals_per_s"],
+                                  "frac": rate / pb["bound_draw_evals_per_s"]}
+            line["fp32_pipe_frac"] = rate * shared_fp32_flops(d, grad, active) / fp32_peak
+        res["adj" if grad else "fwd"] = line
         plan.close()
     res["adjoint_overhead"] = res["fwd"]["draw_evals_per_s"] / res["adj"]["draw_evals_per_s"]
     res["active_fraction"] = active
@@ -1272,10 +1281,14 @@ def run_case(case):
             pkg.mc_smooth_argmax(ctx, v, S, G, G, bandwidth=3.0, degree=2)
         ctx.sync_status()
         return
-    if case in ("c2-shared", "c2-shared-full"):
+    if case in ("c2-shared", "c2-shared-full", "c5-shared"):
         # two scenarios of the d=3 grid (2 x 4096 designs, one stream each),
-        # or the whole grid of the timed step, 1e6 draws
-        prob = workloads.c2(n_scen=2 if case == "c2-shared" else 16, n_draws=1_000_000)
+        # or the whole grid of the timed step, 1e6 draws; or the d=20 grid
+        # (4096 designs), 5e5 draws
+        if case == "c5-shared":
+            prob = workloads.c5(n_draws=500_000)
+        else:
+            prob = workloads.c2(n_scen=2 if case == "c2-shared" else 16, n_draws=1_000_000)
         dp = pkg.DeviceProblem.from_workload(prob)
         jac = torch.as_tensor(prob.jac_packed(), dtype=torch.float64, device="cuda")
         fwd = pkg.Plan(ctx, dp, shared=True)

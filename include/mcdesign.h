@@ -112,9 +112,14 @@ mcd_status mcd_sync_status(mcd_ctx* ctx, mcd_stream stream);
 
 /* MCD_PLAN_SHARED: designs with equal (design_scen, key, draw_begin, n_draws)
  * see the same draws (common random numbers).  Groups of at least
- * MCD_SHARED_MIN such designs are evaluated by the shared-draw kernel, which
- * makes each draw once per block and tests it against every design of the
- * group: hit counts are bit-identical to the per-design kernel, the
+ * MCD_SHARED_MIN such designs make each draw once for many of them.  Gradient
+ * plans, and estimates of small groups, test a draw against every design of the
+ * group (or, for large gradient launches at some dimensions, against the box of
+ * 32 designs first).  Estimates of groups whose predicted time is less that way
+ * reduce each draw to its ranks among the group's thresholds instead; such a
+ * plan holds the ranks of a round (at most 64 MB) and the sorted thresholds
+ * (6 bytes per design and coordinate, for at most 256 groups at once) beside its
+ * tables.  Either way hit counts are bit-identical to the per-design kernel, the
  * likelihood-ratio sums equal up to FP32 rounding.  The sigmoid sums skip,
  * warp by warp, the draws whose every contribution is zero or below 3e-8
  * (no design of the warp within 25 h / log2(e) of the region's boundary in

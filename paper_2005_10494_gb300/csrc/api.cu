@@ -1245,7 +1245,7 @@ mcd_status mcd_plan_config(const mcd_plan* plan, int32_t d, int32_t* threads, in
             const int batch = rank_batch(d, l.words, &th);
             if (threads) *threads = th;
             if (tile_draws) *tile_draws = batch;
-            if (blocks_per_sm) *blocks_per_sm = 1;
+            if (blocks_per_sm) *blocks_per_sm = 1;       // its 512 threads hold 128 registers each
             return MCD_OK;
         }
         return MCD_EINVAL;

@@ -25,7 +25,7 @@
 // Measured on a d=3 grid (4 scenarios x 4096 designs x 1e6 draws): sort 30 us,
 // draws 51 us, count 328 us; the kernel that tests every design against every
 // draw takes 2.53 ms.  The count kernel is bound by shared memory (19 wavefronts
-// a warp step of 8 draws x 512 designs, 63 % of the pipe busy) and the latency
+// a warp step of 8 draws x 512 designs, 65 % of the pipe busy) and the latency
 // of its loads at 16 warps per SM; 24 or 20 warps (768, 640 threads) need the
 // counters in fewer planes and spill, and measured the same or 6 % slower.
 #pragma once

@@ -61,8 +61,9 @@ __device__ inline int basis(double dx, double dy, int degree, bool two_d, double
 // A thread per entry of the normal matrix M sums over the window, the
 // elimination takes a row per thread, and a thread per tap writes the stencil;
 // every entry sees its operations in the order of the sequential solve.  One
-// thread per class pair spent 116 us in chains of FP64 operations, whatever the
-// grid; FP64 latency of one such chain per pivot is what is left.
+// thread per class pair spent 116 us in chains of FP64 operations (2-D, reach 2,
+// 81 pairs, any grid; a line's nine small classes took little and gained nothing);
+// FP64 latency of one such chain per pivot is what is left.
 constexpr int kWeightThreads = 64;
 __global__ void __launch_bounds__(kWeightThreads) weights_kernel(int R, double bw, int degree, bool two_d, int gx, int gy,
                                                                  double* w64, float* w32, DevStatus* status) {
