@@ -83,15 +83,15 @@ struct RankLaunch {
 // groups in either path.  The shared-draw kernel makes its draws once per chunk
 // and tests them in rounds of 256 designs; the ranked path makes them once per
 // family, or-s words of 32 designs, builds rows per chunk, sorts, and runs its three
-// kernels once for every 256 families.  The coefficients are a least-squares fit
-// (90 % of the cases within 35 %) to 668 forward plans of d = 1..20, 1..1500 groups,
-// 32..6000 designs and 12e3..1.5e6 draws in both paths.  Predicted 15 % ahead, the
-// ranked path was slower in one of them (d = 5, 32 groups of 100 x 16k: 90, 100): one
-// group of d = 3, 32 x 1e6 takes 89 us there and 66 ranked, 4096 x 50k 75 and 81; d = 1,
-// 32 groups of 700 x 16k 58 and 84, 300 of 100 x 16k 165 and 188; d = 10, 4096 x 16k 106 and
-// 94.  A line through d x draws x rounds (1.25e6) left calls of 50 to 190 us up to
-// 30 % slower than they had been.
-constexpr double kRankMargin = 1.15;
+// kernels once for every 256 families.  The coefficients are least-squares fits
+// (90 % of the cases within 15 % and 20 %) to 630 forward plans of d = 1..20, 1..1500
+// groups, 32..6000 designs and 16e3..1.5e6 draws in both paths.  With the ranked path
+// predicted 8 % ahead, it was slower than the direct kernel in 7 of them and the direct
+// kernel slower than it by over 3 % in 38: one group of d = 3, 32 x 1e6 takes 89 us there
+// and 66 ranked, 4096 x 50k 75 and 81; d = 1, 32 groups of 700 x 16k 58 and 84, 300 of
+// 100 x 16k 165 and 188; d = 10, 4096 x 16k 89 and 94.  A line through
+// d x draws x rounds (1.25e6) left calls of 50 to 190 us up to 30 % slower.
+constexpr double kRankMargin = 1.08;
 constexpr int kRankFamilies = 256;              // families of one round (their thresholds: 74 KB each at d=3)
 constexpr uint64_t kRankMinDraws = 16384;       // groups of few draws do not pay for their rows
 
@@ -99,16 +99,17 @@ class RankCost {
 public:
     void add(int d, size_t designs, uint64_t draws) {
         const double n = 1e-6 * static_cast<double>(draws);
+        d_ = d;
         const size_t cap = static_cast<size_t>(kSharedThreads) * shared_designs_per_thread(d, false);
         const size_t nch = (designs + cap - 1) / cap, per = (designs + nch - 1) / nch;
         const double rounds = static_cast<double>((per + kSharedThreads - 1) / kSharedThreads);
-        direct_ += static_cast<double>(nch) * n * (6.4 + 0.843 * d * d + 13.6 * rounds * d);
+        direct_ += static_cast<double>(nch) * n * (9.87 + 1.78 * d + 0.104 * d * d + 14.5 * rounds * d);
         const size_t fam = static_cast<size_t>(rank_family(d));
         for (size_t c = 0; c < designs; c += fam) {
             const int cnt = static_cast<int>(std::min(fam, designs - c)), w = rank_words(d, cnt);
             const double chunks = (cnt + 32 * w - 1) / (32 * w);
             const double rows = ((d + 32 / w - 1) / (32 / w)) * (32.0 * w + 1.0) / 256.0;   // of one chunk
-            ranked_ += n * (2.73 + 2.31 * d + 0.204 * d * d + 0.26 * d * w * chunks);
+            ranked_ += n * (4.37 + 2.83 * d + 0.0293 * d * d + 0.28 * d * w * chunks);
             rows_ += rows * chunks;
             most_rows_ = std::max(most_rows_, rows);
             sorts_ += d;
@@ -121,17 +122,17 @@ public:
         int keys = 32;
         while (keys < most_keys_) keys <<= 1;
         const int further = (classes_ & (classes_ - 1)) == 0 ? 0 : classes_ == 28 ? 2 : 1;   // words 4, 8, 16
-        const double t = 56.0 + ranked_ + 5.46 * std::max(most_rows_, rows_ / sms) +
-                         11.8 * static_cast<double>((sorts_ + sms - 1) / sms) * keys / kRankMaxFamily +
-                         95.3 * static_cast<double>((families_ - 1) / kRankFamilies) +
+        const double t = 43.2 + 2.88 * d_ + ranked_ + 1.22 * std::max(most_rows_, rows_ / sms) +
+                         27.9 * static_cast<double>((sorts_ + sms - 1) / sms) * keys / kRankMaxFamily +
+                         90.8 * static_cast<double>((families_ - 1) / kRankFamilies) +
                          25.0 * further;                 // three more launches for each further class of families
-        return t * kRankMargin < 38.5 + direct_;
+        return t * kRankMargin < 21.3 + 2.71 * d_ + direct_;
     }
 
 private:
     double direct_ = 0.0, ranked_ = 0.0, rows_ = 0.0, most_rows_ = 0.0;
     int64_t sorts_ = 0, families_ = 0;
-    int most_keys_ = 0, classes_ = 0;
+    int d_ = 0, most_keys_ = 0, classes_ = 0;
 };
 
 // Blocks per SM for which the tiles of shared draws of a gradient plan are sized.

@@ -65,7 +65,7 @@ RANKED = [
     (10, [(2049, 60_000), (40, 90_001)], 1),
     (13, [(200, 300_001)], 3),
     (17, [(257, 150_001)], 1),
-    (20, [(1025, 40_001), (33, 40_000)], 9),
+    (20, [(1025, 50_001), (33, 50_000)], 9),
     (20, [(32, 1_900_003), (40, 700_001)], 6),
     (4, [(33, 9_000_001), (64, 100_001)], 3),
     (3, [(33, 40_003)] * 300, 1),
